@@ -211,6 +211,7 @@ bool kinetic_skips_deep(const Geom& g);  // learned path: the pass skips deep CT
 bool kinetic_linear_slice(const Geom& g);
 // dvm_linmom.cu (3D windowed HOFKS)
 int linear_moment_arrays();
+bool linear_moments_fit(const Geom& g);  // the grid is within the launch limits of its passes
 int launch_linear_moments(const Geom& g, const DevPtrs& p, cudaStream_t s);  // kernels launched
 void linear_moments_prepare();
 

@@ -414,8 +414,12 @@ void launch_generic(const Geom& g, const DevPtrs& p, cudaStream_t s) {
 // with at least half-filled columns runs 2; per cell against it: 200^2 x 21^2
 // HOFKS 245 against 141 us, 60^3 x 13^3 5.2 against 1.82 ms, implosion 300^2 x
 // 36^2 (p = 2) 1.14 against 0.62 ms, FP64 256^2 x 32^2 5.06 against 3.85 ms.
+// 3D HOFKS without the learned path runs 1 only with the linear-term slice (its
+// single-quadratic form leaves these moments out): beyond the slice's launch
+// limits it is 2 or 0.
 static int kernel_of(const Geom& g) {
-  const bool w = window_eligible(g), sh = shared_eligible(g);
+  const bool sh = shared_eligible(g);
+  const bool w = window_eligible(g) && (g.d == 2 || g.scheme == DVM_FKS || g.learn || linear_moments_fit(g));
   if (!w || !sh) return w ? 1 : (sh ? 2 : 0);
   if (g.learn) return 1;
   if (g.scheme == DVM_FKS) return 2;
@@ -461,7 +465,7 @@ bool kinetic_linear_slice(const Geom& g) {
   if (g.d != 3 || g.scheme == DVM_FKS || g.p != 1 || !kinetic_is_windowed(g)) return false;
   for (int i = 0; i < 3; ++i)
     if (g.bc[i] != DVM_BC_PERIODIC) return false;
-  return g.nx[2] <= 3000 && g.nx[1] <= 65535;
+  return linear_moments_fit(g);
 }
 
 void launch_gauss_tables(const Geom& g, const DevPtrs& p, const double* prm, cudaStream_t s) {

@@ -377,6 +377,11 @@ int linear_moment_arrays() {
   return T.nx + T.ny;
 }
 
+// The y pass takes a grid z per z plane and x-sum, the z pass one per y.
+bool linear_moments_fit(const Geom& g) {
+  return (long long)g.nx[2] * tables().y.nin <= 65535 && g.nx[1] <= 65535;
+}
+
 // B into the last split of the partial sums (see the top of this file); with
 // the learned path (whose window pass sums both parts itself) that split is
 // zero.  Returns the kernels launched.
