@@ -163,7 +163,8 @@ bool shared_eligible(const Geom& g) {
 // the partial sums' share of the traffic; where the tiles alone fill the chip
 // many times over, c <= 4 (their memory); 2D periodic HOFKS c <= 6 p, for the step
 // waits for the 1/p as many Euler sub-steps beside it and the CTAs take their
-// SMs.  Step of the implosion 200^2 x 30^2, c = 5, 8, 15, 30: 339, 287, 253, 260
+// SMs; 2D FP32 at least pairs / kShRun, for a split's sums are FP32 and the splits
+// are added in FP64.  Step of the implosion 200^2 x 30^2, c = 5, 8, 15, 30: 339, 287, 253, 260
 // us; FKS 200^2 x 20^2, c = 4, 7, 12: 65, 54, 63 us; FP64 HOFKS 100^2 x 40^2,
 // c = 10, 20, 40: 1471, 1163, 1124 us; HOFKS 64^2 x 25^2, c = 6, 12, 25: 126,
 // 135, 138 us.
@@ -174,9 +175,11 @@ int shared_splits(const Geom& g, int sms) {
   const int per_sm = f64 ? 2 : (fks ? 4 : 3);
   int most = tiles >= 8LL * sms ? 4 : kMaxSplits;
   if (g.d == 2 && !fks && !even) most = std::min(most, 6 * g.p);
-  int best = 1;
+  const int least = g.d == 2 && !f64 ? (pairs + kShRun - 1) / kShRun : 1;
+  static_assert(kMaxV1 <= kMaxSplits * kShRun, "every x axis can be split into short runs");
+  int best = least;
   double cost = 1e30;
-  for (int c = 1; c <= most && c <= pairs; ++c) {
+  for (int c = least; c <= std::max(most, least) && c <= pairs; ++c) {
     const long long slots = (long long)sms * per_sm, ctas = tiles * c, full = ctas / slots, rest = ctas % slots;
     const double k = (double)((rest + sms - 1) / sms) / per_sm;
     const double waves = even ? (double)ctas / slots + 0.5 : (double)full + (rest ? pow(k, 0.3) : 0.0);
