@@ -207,19 +207,31 @@ int dvm_load(dvm_handle* h, const void* buf, size_t bytes);
 /* Kernel launches enqueued by one time step (the captured graph's nodes). */
 int dvm_launches_per_step(dvm_handle* h, int* launches);
 
-/* Which kinetic-pass kernel the handle's steps run (chosen at dvm_create
- * from the grid, precision and boundaries): DVM_KPASS_GENERIC (1D and FP64
- * storage, and boxes flat in y: one thread per cell; 2D/3D FP64 shares folded
- * source rows per CTA) or DVM_KPASS_WINDOW (FP32/BF16 storage, 2D/3D: windows
- * of source rows that slide along the velocity, per thread or shared by the
- * CTA). */
+/* Which arithmetic the handle's kinetic pass has (from the grid, precision and
+ * boundaries): DVM_KPASS_GENERIC (1D and FP64 storage, and boxes flat in y) or
+ * DVM_KPASS_WINDOW (FP32/BF16 storage, 2D/3D: parameters of the source rows
+ * folded per velocity pair).  dvm_kinetic_route says which kernel it is. */
 enum { DVM_KPASS_GENERIC = 0, DVM_KPASS_WINDOW = 1 };
 int dvm_kinetic_kernel(const dvm_handle* h, int* kind);
 
-/* Velocity chunks of the kinetic pass (chosen at dvm_create from the grid and
- * the SM count): the velocity loop of every target cell is split over this
- * many CTAs, each writing its own FP64 partial moment sums, which the
- * end-of-step kernel adds (Eq. DM summed in parts).  1 = no split. */
+/* The kernel that the handle's steps run now (switching the learned path on or
+ * off may change it, and the splits with it) and, for DVM_ROUTE_SHARED, the
+ * folded source rows a CTA holds (else 0):
+ *   DVM_ROUTE_CELL    one thread per cell, any configuration
+ *   DVM_ROUTE_WINDOW  per-thread windows of source rows (FP32/BF16, periodic
+ *                     2D/3D, p = 1)
+ *   DVM_ROUTE_SHARED  source rows folded once per CTA (2D/3D, every storage)
+ *   DVM_ROUTE_TILE    the configured 3D FP32 shapes
+ * dvm_plan_route: what dvm_create would choose for cfg; host only, as dvm_plan. */
+enum { DVM_ROUTE_CELL = 0, DVM_ROUTE_WINDOW = 1, DVM_ROUTE_SHARED = 2, DVM_ROUTE_TILE = 3 };
+int dvm_kinetic_route(const dvm_handle* h, int* route, int* rows);
+int dvm_plan_route(const dvm_config* cfg, int* route, int* rows);
+
+/* Velocity chunks of the kinetic pass (from the grid and the SM count; other
+ * ones while the learned path is on, where it runs another kernel): the
+ * velocity loop of every target cell is split over this many CTAs, each writing
+ * its own FP64 partial moment sums, which the end-of-step kernel adds (Eq. DM
+ * summed in parts).  1 = no split. */
 int dvm_kinetic_splits(const dvm_handle* h, int* splits);
 
 /* The kinetic-pass plan dvm_create would choose for cfg, without creating

@@ -887,6 +887,22 @@ int dvm_kinetic_kernel(const dvm_handle* h, int* kind) {
   return 0;
 }
 
+int dvm_kinetic_route(const dvm_handle* h, int* route, int* rows) {
+  if (!h || !route || !rows) return DVM_ERR_ARG;
+  *route = kinetic_route(h->g, rows);
+  return 0;
+}
+
+int dvm_plan_route(const dvm_config* cfg, int* route, int* rows) {
+  Geom g;
+  std::string msg;
+  const int rc = make_geom(cfg, &g, &msg);
+  if (rc) return rc;
+  if (!route || !rows) return DVM_ERR_ARG;
+  *route = kinetic_route(g, rows);
+  return 0;
+}
+
 int dvm_kinetic_splits(const dvm_handle* h, int* splits) {
   if (!h || !splits) return DVM_ERR_ARG;
   *splits = h->g.nsplit - h->g.lin_slice;

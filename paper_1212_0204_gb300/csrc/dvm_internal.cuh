@@ -199,14 +199,17 @@ void launch_gauss_tables(const Geom& g, const DevPtrs& p, const double* prm, cud
 bool launch_window_fixed(const Geom& g, const DevPtrs& p, int splits, cudaStream_t s, bool prepare);
 // 3D FP32 HOFKS at a shape the tile kernel is compiled for (dvm_kinetic_shapes.cu)
 bool tile3_shape(const Geom& g);
+bool fixed_shapes_on();  // (DVM_FIXED_SHAPES)
 // the pass with CTA-shared source rows (dvm_kinetic_shared.cu)
 bool shared_eligible(const Geom& g);
 int shared_splits(const Geom& g, int sms);
+int shared_rows(const Geom& g);  // folded rows per CTA
 void shared_prepare(const Geom& g);
 void launch_shared(const Geom& g, const DevPtrs& p, int splits, cudaStream_t s);
 void kinetic_pass_prepare(const Geom& g);
 int kinetic_pass_splits(const Geom& g);
 bool kinetic_is_windowed(const Geom& g);
+int kinetic_route(const Geom& g, int* rows);  // DVM_ROUTE_*; folded rows of the shared pass
 bool kinetic_skips_deep(const Geom& g);  // learned path: the pass skips deep CTAs
 bool kinetic_linear_slice(const Geom& g);
 // dvm_linmom.cu (3D windowed HOFKS)

@@ -456,6 +456,14 @@ void kinetic_pass_prepare(const Geom& g) {
 
 bool kinetic_is_windowed(const Geom& g) { return g.precision != DVM_F64 && kernel_of(g) != 0 && !getenv_generic(); }
 
+int kinetic_route(const Geom& g, int* rows) {
+  const int k = getenv_generic() ? 0 : kernel_of(g);
+  *rows = k == 2 ? shared_rows(g) : 0;
+  if (k == 2) return DVM_ROUTE_SHARED;
+  if (k == 0) return DVM_ROUTE_CELL;
+  return tile3_shape(g) && !g.learn && fixed_shapes_on() && window_async(3) ? DVM_ROUTE_TILE : DVM_ROUTE_WINDOW;
+}
+
 // (the per-thread windows skip CTAs whose targets are all deep)
 bool kinetic_skips_deep(const Geom& g) { return kernel_of(g) == 1 && !getenv_generic(); }
 

@@ -69,10 +69,14 @@ bool tile3_shape(const Geom& g) {
 
 // DVM_FIXED_SHAPES=0 runs the runtime-extent kernel for every shape (for
 // comparison runs and the test that both give the same result).
+bool fixed_shapes_on() {
+  const char* e = getenv("DVM_FIXED_SHAPES");
+  return !(e && e[0] == '0');
+}
+
 bool launch_window_fixed(const Geom& g, const DevPtrs& p, int splits, cudaStream_t s, bool prepare) {
   if (g.precision == DVM_F64 || g.scheme == DVM_FKS) return false;
-  const char* e = getenv("DVM_FIXED_SHAPES");
-  if (e && e[0] == '0' && !prepare) return false;
+  if (!fixed_shapes_on() && !prepare) return false;
   if (g.precision == DVM_BF16S) {
     // BF16 storage: the 2D 256^2 / 512^2 and 3D 64^3 / 96^3 shapes, no learned path
     if (g.learn) return false;

@@ -189,6 +189,8 @@ int shared_splits(const Geom& g, int sms) {
   return best;
 }
 
+int shared_rows(const Geom& g) { return shape_of(g, 1).rows; }
+
 void shared_prepare(const Geom& g) {
   DevPtrs none{};
   // the forms with and without the learned path

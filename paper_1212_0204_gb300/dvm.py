@@ -29,7 +29,7 @@ EXPORTS = [
     "dvm_workspace_bytes", "dvm_create", "dvm_destroy", "dvm_set_stream", "dvm_last_error",
     "dvm_set_state_moments", "dvm_set_state_primitive", "dvm_step", "dvm_step_async",
     "dvm_sync_status", "dvm_moments", "dvm_moments_async", "dvm_moments_wait", "dvm_get_f", "dvm_last_parts", "dvm_info", "dvm_offsets",
-    "dvm_save", "dvm_load", "dvm_launches_per_step", "dvm_kinetic_kernel", "dvm_kinetic_splits", "dvm_plan", "dvm_profile_begin",
+    "dvm_save", "dvm_load", "dvm_launches_per_step", "dvm_kinetic_kernel", "dvm_kinetic_route", "dvm_plan_route", "dvm_kinetic_splits", "dvm_plan", "dvm_profile_begin",
     "dvm_profile_end",
     "dvm_equilibrium_noalloc", "dvm_selftest_timeout",
     "dvm_batch_create", "dvm_batch_destroy", "dvm_batch_last_error", "dvm_batch_sizes",
@@ -127,6 +127,8 @@ def lib():
         L.dvm_load.argtypes = [vp, vp, C.c_size_t]
         L.dvm_launches_per_step.argtypes = [vp, C.POINTER(C.c_int)]
         L.dvm_kinetic_kernel.argtypes = [vp, C.POINTER(C.c_int)]
+        L.dvm_kinetic_route.argtypes = [vp, C.POINTER(C.c_int), C.POINTER(C.c_int)]
+        L.dvm_plan_route.argtypes = [C.POINTER(_Config), C.POINTER(C.c_int), C.POINTER(C.c_int)]
         L.dvm_kinetic_splits.argtypes = [vp, C.POINTER(C.c_int)]
         L.dvm_plan.argtypes = [C.POINTER(_Config), C.POINTER(C.c_int), C.POINTER(C.c_int)]
         L.dvm_profile_begin.argtypes = [vp]
@@ -245,6 +247,19 @@ def plan(cfg) -> tuple:
     if rc:
         raise DvmError(rc, "invalid configuration")
     return ("generic", "window")[kind.value], splits.value
+
+
+ROUTES = ("cell", "window", "shared", "tile")
+
+
+def plan_route(cfg) -> tuple:
+    """(kernel of the kinetic pass, folded source rows per CTA) that dvm_create would choose
+    for cfg (dvm_plan_route; host only)."""
+    route, rows = C.c_int(), C.c_int()
+    rc = lib().dvm_plan_route(C.byref(cfg), C.byref(route), C.byref(rows))
+    if rc:
+        raise DvmError(rc, "invalid configuration")
+    return ROUTES[route.value], rows.value
 
 
 def workspace_bytes(cfg) -> int:
@@ -415,10 +430,18 @@ class Solver:
         return n.value
 
     def kinetic_kernel(self) -> str:
-        """'generic' or 'window': the kinetic-pass kernel of this handle."""
+        """'generic' or 'window': the arithmetic of this handle's kinetic pass (kinetic_route
+        names the kernel)."""
         k = C.c_int()
         self._check(lib().dvm_kinetic_kernel(self._h, C.byref(k)))
         return ("generic", "window")[k.value]
+
+    def kinetic_route(self) -> tuple:
+        """(kernel that the steps run now: 'cell', 'window', 'shared' or 'tile'; folded source
+        rows per CTA of 'shared', else 0)."""
+        route, rows = C.c_int(), C.c_int()
+        self._check(lib().dvm_kinetic_route(self._h, C.byref(route), C.byref(rows)))
+        return ROUTES[route.value], rows.value
 
     def kinetic_splits(self) -> int:
         """Velocity chunks of the kinetic pass (CTAs per target tile)."""
