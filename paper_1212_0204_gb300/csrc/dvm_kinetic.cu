@@ -402,18 +402,36 @@ void launch_generic(const Geom& g, const DevPtrs& p, cudaStream_t s) {
 
 }  // namespace
 
+// Where both the per-thread windows and the shared rows can run (periodic, p = 1,
+// velocity counts a multiple of the windows'), per step in us, windows / shared.
+// 2D: FKS shared (256^2 x 32^2 173 / 158, 200^2 x 24^2 114 / 70); HOFKS windows, for
+// the shared rows' CTAs leave the Euler sub-steps beside them less room (256^2 x
+// 32^2 203 / 271, 512^2 x 32^2 873 / 991).
+// 3D: by the share of useful lanes, N_x of 32-wide rows against N_y of 16-row
+// columns.  Shared where its share is larger by a tenth (40^3 x 16^3 HOFKS 1726 /
+// 1146, 48^3 x 16^3 2028 / 1661, 80^3 x 20^3 13250 / 11020, 100^3 x 12^3 FKS 6453 /
+// 4310).  Alike and ragged, windows (60^3 x 20^3 HOFKS 4568 / 5201, 90^3 x 24^3 25350 /
+// 31030, FKS 23310 / 29870; 88^3 x 16^3 8202 / 8298, FKS 6950 / 7421).  Whole tiles,
+// shared from 16 velocities along y up (32^3 x 16^3 561 / 490, 64^3 x 20^3 5020 / 4940;
+// 64^3 x 12^3 1462 / 1585, BF16 FKS 1094 / 1146), FP32 FKS always (64^3 x 12^3 1063 /
+// 1026).  Small grids windows (24^3 x 12^3 248 / 290, FKS 104 / 124).  BF16 HOFKS and the
+// tile kernel's shapes stay with 1.
+static bool shared_faster(const Geom& g) {
+  const bool fks = g.scheme == DVM_FKS, f32 = g.precision == DVM_F32;
+  if (g.d == 2) return fks;
+  if (!fks && (!f32 || tile3_shape(g))) return false;
+  if (g.nc < (1 << 14)) return false;
+  const long long bx = (g.nx[0] + 31LL) / 32 * 32, by = (g.nx[1] + 15LL) / 16 * 16;
+  if (10 * g.nx[1] * bx >= 11 * g.nx[0] * by) return true;
+  return g.nx[0] == bx && g.nx[1] == by && (g.nv[1] >= 16 || (fks && f32));
+}
+
 // Which kernel of the pass: 0 one thread per cell, 1 the per-thread windows
 // (and the kernels compiled for the configured shapes), 2 the CTA-shared rows.
-// Where both 1 and 2 can run (periodic, p = 1, velocity counts a multiple of
-// the windows'), per step: FKS 2 (256^2 x 32^2 162 against 174 us, 64^3 x 12^3
-// 976 against 1068); 3D FP32 HOFKS outside the configured shapes 2 (48^3 x 16^3
-// 1.68 against 2.06 ms, 64^3 x 16^3 2.84 against 2.89); 3D BF16 1 (64^3 x 16^3
-// 2.95 against 3.09 ms); 2D HOFKS 1 (its CTAs leave the Euler sub-steps beside
-// it more room: 100^2 x 16^2 87 against 97 us, 256^2 x 32^2 229 against 290).
-// The learned path keeps 1, which skips CTAs of flagged cells.  Everything else
-// with at least half-filled columns runs 2; per cell against it: 200^2 x 21^2
-// HOFKS 245 against 141 us, 60^3 x 13^3 5.2 against 1.82 ms, implosion 300^2 x
-// 36^2 (p = 2) 1.14 against 0.62 ms, FP64 256^2 x 32^2 5.06 against 3.85 ms.
+// The learned path keeps 1, which skips CTAs of flagged cells.  What 1 does not
+// take runs 2 where its columns are at least half filled; per cell against it:
+// 200^2 x 21^2 HOFKS 245 against 141 us, 60^3 x 13^3 5.2 against 1.82 ms, implosion
+// 300^2 x 36^2 (p = 2) 1.14 against 0.62 ms, FP64 256^2 x 32^2 5.06 against 3.85 ms.
 // 3D HOFKS without the learned path runs 1 only with the linear-term slice (its
 // single-quadratic form leaves these moments out): beyond the slice's launch
 // limits it is 2 or 0.
@@ -421,10 +439,7 @@ static int kernel_of(const Geom& g) {
   const bool sh = shared_eligible(g);
   const bool w = window_eligible(g) && (g.d == 2 || g.scheme == DVM_FKS || g.learn || linear_moments_fit(g));
   if (!w || !sh) return w ? 1 : (sh ? 2 : 0);
-  if (g.learn) return 1;
-  if (g.scheme == DVM_FKS) return 2;
-  if (g.d == 2) return 1;
-  return g.precision == DVM_F32 && !tile3_shape(g) ? 2 : 1;
+  return !g.learn && shared_faster(g) ? 2 : 1;
 }
 
 // Velocity chunks; of the per-cell pass enough blocks for several waves on 152

@@ -48,3 +48,21 @@ def test_kernels_of_the_storage_tiers():
     assert route((64, 64, 64), (24, 24, 24), dvm.F32, dvm.HOFKS) == ("tile", 0)
     assert route((64, 64, 64), (24, 24, 24), dvm.BF16S, dvm.HOFKS) == ("window", 0)
     assert route((4, 8, 3856), (8, 8, 6), dvm.F32, dvm.HOFKS) == ("cell", 0)
+
+
+@pytest.mark.parametrize("n,nv,scheme,precision,want", [
+    # where both kernels can run in 3D: by the share of useful lanes of either
+    (40, 16, dvm.HOFKS, dvm.F32, "shared"),
+    (60, 20, dvm.HOFKS, dvm.F32, "window"),
+    (60, 20, dvm.FKS, dvm.F32, "window"),
+    (90, 24, dvm.FKS, dvm.BF16S, "window"),
+    (100, 12, dvm.FKS, dvm.F32, "shared"),
+    (64, 12, dvm.FKS, dvm.F32, "shared"),
+    (64, 12, dvm.FKS, dvm.BF16S, "window"),
+    (64, 12, dvm.HOFKS, dvm.F32, "window"),
+    (64, 16, dvm.HOFKS, dvm.F32, "shared"),
+    (24, 12, dvm.FKS, dvm.F32, "window"),
+    (48, 16, dvm.HOFKS, dvm.BF16S, "window"),
+])
+def test_kernels_of_3d_boxes(n, nv, scheme, precision, want):
+    assert route((n,) * 3, (nv,) * 3, precision, scheme)[0] == want
