@@ -487,6 +487,13 @@ int dvm_equilibrium_noalloc(const dvm_config* cfg, const double* U, double* f,
 enum { DVM_SELFTEST_GRID_BARRIER = 0, DVM_SELFTEST_MBARRIER = 1 };
 int dvm_selftest_timeout(int which, void* cuda_stream, int* status);
 
+/* The FP64 arithmetic of the Euler sub-steps that does not use the compiler's
+ * division and square root, on n values of device arrays: out = 1 / a, a / b,
+ * sqrt(a), or half the limited slope of two halved differences, a b / (a + b) if
+ * both have one sign, else 0. */
+enum { DVM_SELFTEST_RCP = 0, DVM_SELFTEST_QUOT = 1, DVM_SELFTEST_SQRT = 2, DVM_SELFTEST_HALF_SLOPE = 3 };
+int dvm_selftest_fp64(int which, long long n, const double* a, const double* b, double* out, void* cuda_stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -92,8 +92,8 @@ __global__ void __launch_bounds__(256) k_euler1d(Geom g, DevPtrs p) {
   const int ml = lrank < 0 ? 0 : (int)((long long)(lrank + 1) * nx / C) - (int)((long long)lrank * nx / C);
   double ad = __longlong_as_double((long long)__ldcg(p.aslot));
   const double a0 = ad;
-  // (constant over the sub-steps; the face this thread evaluates)
-  const double rdx = sizeof(TF) == 8 ? rcp64(g.dx) : 0.0;
+  __shared__ TF s_kk;
+  __shared__ int s_flags;  // bit 0: last sub-step, bit 1: no wave
   const int fk = tid / (m + 1), ff = tid - fk * (m + 1);
   double t = 0.0;
   int s = 0;
@@ -101,23 +101,28 @@ __global__ void __launch_bounds__(256) k_euler1d(Geom g, DevPtrs p) {
   cl.sync();  // every CTA runs before its shared memory is written
   for (;; ++s) {
     const int cur = s & 1;
-    // alpha and length of the sub-step (Eq. Time2), by every thread
-    double dtE;
-    if (g.forced_sub > 0) {
-      dtE = g.dt / g.forced_sub;
-      last = s + 1 == g.forced_sub;
-    } else if (!(ad > 0.0)) {
-      if (rank == 0 && tid == 0) set_status(p.status, DVM_ERR_NONPHYSICAL);
-      return;
-    } else {
-      const double cfl = sizeof(TF) == 8 ? quot64(0.5 * g.dx, ad, rcp64(ad))
-                                         : (double)__fdiv_rn(0.5f * (float)g.dx, (float)ad);
-      const double rem = __dsub_rn(g.dt, t);
-      last = cfl >= rem;
-      dtE = last ? rem : cfl;
+    // length of the sub-step (Eq. Time2) by the last warp, which has no cells,
+    // while the others form the split fluxes
+    if (tid == NT - 1) {
+      double dtE = 0.0;
+      int flags = 0;
+      if (g.forced_sub > 0) {
+        dtE = g.dt / g.forced_sub;
+        flags = s + 1 == g.forced_sub;
+      } else if (!(ad > 0.0)) {
+        flags = 2;
+        if (rank == 0) set_status(p.status, DVM_ERR_NONPHYSICAL);
+      } else {
+        const double cfl = sizeof(TF) == 8 ? __ddiv_rn(__dmul_rn(0.5, g.dx), ad)
+                                           : (double)__fdiv_rn(0.5f * (float)g.dx, (float)ad);
+        const double rem = __dsub_rn(g.dt, t);
+        flags = cfl >= rem;
+        dtE = flags ? rem : cfl;
+      }
+      t = __dadd_rn(t, dtE);
+      s_kk = sizeof(TF) == 8 ? (TF)(dtE / g.dx) : (TF)((float)dtE / (float)g.dx);
+      s_flags = flags;
     }
-    t = __dadd_rn(t, dtE);
-    const TF kk = sizeof(TF) == 8 ? (TF)quot64(dtE, g.dx, rdx) : (TF)((float)dtE / (float)g.dx);
     const TF al = (TF)ad;
     if (tid < m + 4) {
       const int i = tid;
@@ -129,6 +134,9 @@ __global__ void __launch_bounds__(256) k_euler1d(Geom g, DevPtrs p) {
       for (int k = 0; k < NM; ++k) s_g[k][i] = gp[k], s_g[NM + k][i] = gm[k];
     }
     __syncthreads();
+    if (s_flags & 2) return;
+    last = s_flags & 1;
+    const TF kk = s_kk;
     // psi between cells f - 1 and f (entries f + 1 and f + 2)
     if (fk < NM) {
       const int k = fk, f = ff;

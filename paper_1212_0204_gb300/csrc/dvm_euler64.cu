@@ -87,12 +87,12 @@ __global__ void __launch_bounds__(kE64Threads) k_euler64(Geom g, DevPtrs p, Tile
         flags = 2;
         if (blockIdx.x == 0) set_status(p.status, DVM_ERR_NONPHYSICAL);
       } else {
-        const double cfl = quot64(0.5 * g.dx, asum, rcp64(asum)), rem = __dsub_rn(g.dt, t);
+        const double cfl = __ddiv_rn(__dmul_rn(0.5, g.dx), asum), rem = __dsub_rn(g.dt, t);
         flags = cfl >= rem;
         dtE = flags ? rem : cfl;
       }
       t = __dadd_rn(t, dtE);
-      s_t[0] = ad[0], s_t[1] = ad[1], s_t[2] = quot64(dtE, g.dx, rcp64(g.dx));
+      s_t[0] = ad[0], s_t[1] = ad[1], s_t[2] = dtE / g.dx;
       s_flags = flags;
     }
     double amax[2] = {0.0, 0.0};

@@ -6,6 +6,8 @@
 //     one of two blocks leaving without arriving (about 1 s);
 //   DVM_SELFTEST_MBARRIER: the mbarrier wait of the tensor-core kernels on a
 //     barrier nobody arrives at (about 1 s).
+// dvm_selftest_fp64 applies the FP64 pieces of dvm_euler64.cuh to arrays.
+#include "dvm_euler64.cuh"
 #include "dvm_internal.cuh"
 #include "dvm_math.cuh"
 #include "dvm_tc.cuh"
@@ -28,8 +30,28 @@ __global__ void k_selftest_mbar(int* status) {
   if (threadIdx.x == 0 && !tc::mbar_wait(&mbar, 0)) set_status(status, DVM_ERR_TIMEOUT);
 }
 
+__global__ void k_selftest_fp64(int which, long long n, const double* a, const double* b, double* out) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double x = a[i], y = b[i];
+  if (which == DVM_SELFTEST_RCP) out[i] = rcp64(x);
+  else if (which == DVM_SELFTEST_QUOT) out[i] = quot64(x, y, rcp64(y));
+  else if (which == DVM_SELFTEST_SQRT) out[i] = sqrt64(x);
+  else out[i] = half_slope<true>(x, y);
+}
+
 }  // namespace
 }  // namespace dvm
+
+extern "C" int dvm_selftest_fp64(int which, long long n, const double* a, const double* b, double* out,
+                                 void* cuda_stream) {
+  using namespace dvm;
+  if (which < DVM_SELFTEST_RCP || which > DVM_SELFTEST_HALF_SLOPE || n < 1 || n > (1LL << 30) || !a || !b || !out)
+    return DVM_ERR_ARG;
+  cudaStream_t s = (cudaStream_t)cuda_stream;
+  k_selftest_fp64<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(which, n, a, b, out);
+  return cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess ? 0 : DVM_ERR_CUDA;
+}
 
 extern "C" int dvm_selftest_timeout(int which, void* cuda_stream, int* status) {
   using namespace dvm;

@@ -23,6 +23,7 @@ PERIODIC, OUTFLOW = 0, 1
 FKS, HOFKS, HOFKS_UNLIMITED, HOFKS_WENO, FKS_STRANG = 0, 1, 2, 3, 4
 F64, F32, BF16S = 0, 1, 2
 SELFTEST_GRID_BARRIER, SELFTEST_MBARRIER = 0, 1
+SELFTEST_RCP, SELFTEST_QUOT, SELFTEST_SQRT, SELFTEST_HALF_SLOPE = 0, 1, 2, 3
 
 # every symbol include/dvm.h declares (checked by the CPU tests)
 EXPORTS = [
@@ -31,7 +32,7 @@ EXPORTS = [
     "dvm_sync_status", "dvm_moments", "dvm_moments_async", "dvm_moments_wait", "dvm_get_f", "dvm_last_parts", "dvm_info", "dvm_offsets",
     "dvm_save", "dvm_load", "dvm_launches_per_step", "dvm_kinetic_kernel", "dvm_kinetic_route", "dvm_plan_route", "dvm_kinetic_splits", "dvm_plan", "dvm_profile_begin",
     "dvm_profile_end",
-    "dvm_equilibrium_noalloc", "dvm_selftest_timeout",
+    "dvm_equilibrium_noalloc", "dvm_selftest_timeout", "dvm_selftest_fp64",
     "dvm_batch_create", "dvm_batch_destroy", "dvm_batch_last_error", "dvm_batch_sizes",
     "dvm_batch_moment_rows",
     "dvm_batch_set_state_moments", "dvm_batch_step", "dvm_batch_step_async",
@@ -135,6 +136,7 @@ def lib():
         L.dvm_profile_end.argtypes = [vp, dp, C.POINTER(C.c_int)]
         L.dvm_equilibrium_noalloc.argtypes = [C.POINTER(_Config), vp, vp, vp]
         L.dvm_selftest_timeout.argtypes = [C.c_int, vp, C.POINTER(C.c_int)]
+        L.dvm_selftest_fp64.argtypes = [C.c_int, C.c_longlong, vp, vp, vp, vp]
         L.dvm_batch_create.argtypes = [C.POINTER(_Config), ip, vp, C.POINTER(vp)]
         L.dvm_batch_destroy.argtypes = [vp]
         L.dvm_batch_destroy.restype = None
@@ -237,6 +239,21 @@ def selftest_timeout(which: int, stream=None) -> int:
     if rc:
         raise DvmError(rc, "selftest launch failed")
     return st.value
+
+
+def selftest_fp64(which: int, a, b):
+    """The FP64 pieces of the Euler sub-steps (dvm_selftest_fp64) on CUDA tensors of doubles."""
+    import torch
+    if not (a.is_cuda and b.is_cuda and a.dtype == b.dtype == torch.float64 and a.shape == b.shape):
+        raise ValueError("two CUDA tensors of float64 of one shape")
+    a, b = a.contiguous(), b.contiguous()
+    out = torch.empty_like(a)
+    stream = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    rc = lib().dvm_selftest_fp64(int(which), a.numel(), C.c_void_p(a.data_ptr()), C.c_void_p(b.data_ptr()),
+                                 C.c_void_p(out.data_ptr()), stream)
+    if rc:
+        raise DvmError(rc, "selftest launch failed")
+    return out
 
 
 def plan(cfg) -> tuple:
