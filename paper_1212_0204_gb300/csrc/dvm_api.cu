@@ -545,6 +545,7 @@ int dvm_create(const dvm_config* cfg, void* workspace, void* cuda_stream, dvm_ha
     h->tau_host[c] = (float)(cfg->tau_field ? cfg->tau_field[c] : cfg->tau);
   h->all_free = all_free;
   h->g.skip_euler = all_free ? 1 : 0;
+  if (h->g.d <= 2 && h->g.precision == DVM_F64) euler64_tile(&h->g);
   h->g.euler_blocks = euler_blocks(h->g);
   // optional cap of the Euler grid (fewer co-resident blocks leave room on
   // every SM for the concurrent kinetic pass)

@@ -250,8 +250,10 @@ __global__ void __launch_bounds__(kE64Threads) k_euler64(Geom g, DevPtrs p, Tile
 
 // The tile whose busiest SM has the fewest FP64 instructions per sub-step, in
 // warps x instructions: states 45 each, faces 24, updates with alpha 90, and
-// 120 a tile for its barriers; at most 100 KB of shared memory.
-Tile64 tile64(const Geom& g, int sms) {
+// 120 a tile for its barriers; at most 100 KB of shared memory.  Up to 4000
+// candidates, so once per handle (searched at every launch, a step outside a graph cost the
+// host 16 us instead of 10).
+Tile64 best_tile64(const Geom& g, int sms) {
   const int nm = g.d + 2;
   auto warps = [](int n) { return (n + 31) / 32; };
   Tile64 best{};
@@ -269,19 +271,23 @@ Tile64 tile64(const Geom& g, int sms) {
   return best;
 }
 
+Tile64 tile64(const Geom& g) {
+  const int tx = g.euler_tile[0], ty = g.euler_tile[1], ntx = (g.nx[0] + tx - 1) / tx;
+  return {tx, ty, ntx, ntx * ((g.nx[1] + ty - 1) / ty)};
+}
+
 template <int D, bool LIMITED>
 cudaError_t launch_t(const Geom& g, const DevPtrs& p, cudaStream_t s, bool prepare, int* blocks, cudaEvent_t started) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const Tile64 T = tile64(g, sms);
+  const Tile64 T = tile64(g);
   const size_t smem = sizeof(double) * smem64(D, T.tx, T.ty);
   auto* k = k_euler64<D, LIMITED>;
   const int items = std::max((D + 2) * ((T.tx + 1) * T.ty + (D == 2 ? T.tx * (T.ty + 1) : 0)), 64);
   const int threads = std::min(kE64Threads, (items + 31) / 32 * 32);
   if (prepare) {
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-    int per_sm = 0;
+    int per_sm = 0, dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
     *blocks = (int)std::min<long long>((long long)sms * std::max(per_sm, 1), T.ntiles);
     return cudaGetLastError();
@@ -305,6 +311,14 @@ cudaError_t launch_t(const Geom& g, const DevPtrs& p, cudaStream_t s, bool prepa
 }
 
 }  // namespace
+
+void euler64_tile(Geom* g) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const Tile64 T = best_tile64(*g, sms);
+  g->euler_tile[0] = T.tx, g->euler_tile[1] = T.ty;
+}
 
 cudaError_t launch_euler64(const Geom& g, const DevPtrs& p, bool limited, cudaStream_t s, bool prepare, int* blocks,
                            cudaEvent_t started) {

@@ -79,6 +79,7 @@ struct Geom {
   long long goff[3];  // first element of dimension i's snapshot (ghost_index)
   int skip_euler;     // every lambda == 1: U_E = 0, no Euler launch
   int euler_blocks;   // grid of the cooperative Euler launch (all co-resident)
+  int euler_tile[2];  // FP64 1D/2D: cells of its tiles (chosen at creation)
   int learn;          // learned regime path on: flagged cells (see dvm_learn.cuh)
 };
 
@@ -184,6 +185,7 @@ bool euler_records_start(const Geom& g);  // launch_euler records `started`
 // dvm_euler32.cu: the 2D sub-steps in FP32 of larger grids
 cudaError_t launch_euler32(const Geom& g, const DevPtrs& p, bool limited, cudaStream_t s, bool prepare, int* blocks);
 // dvm_euler64.cu: the 1D and 2D sub-steps in FP64 (prepare: only the grid size)
+void euler64_tile(Geom* g);
 cudaError_t launch_euler64(const Geom& g, const DevPtrs& p, bool limited, cudaStream_t s, bool prepare, int* blocks,
                            cudaEvent_t started);
 void launch_ghost(const Geom& g, const DevPtrs& p, cudaStream_t s);
