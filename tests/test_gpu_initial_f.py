@@ -78,3 +78,18 @@ def test_initial_f_of_an_fp32_batch():
     b.set_moments(b.pack(U0))
     for i, c in enumerate(cases):
         check(c, U0[i], np.asarray(b.f(i)))
+
+
+@pytest.mark.parametrize("form", [CASES[0], CASES[4], CASES[6]])
+def test_initial_f_below_the_normal_range(form):
+    """Densities of 2^-122: most values are subnormal.  The exponent, -120 to -135, is rounded to
+    half of 2^-17 or 2^-16: 2.6e-6 or 5.3e-6 of a value at most, and values to 2^-150."""
+    case = noisy_case(*form, seed=7)
+    U0 = np.ldexp(conserved(case), -122)
+    orc = oracle.Scheme(grid(case), tau=case.tau)
+    orc.set_moments(U0)
+    s = dvm.Solver.from_case(case, precision=dvm.F32)
+    s.set_moments(U0)
+    f = s.f()
+    fo = orc.f().reshape(f.shape)
+    assert np.linalg.norm(f - fo) <= 5.3e-6 * np.linalg.norm(fo) + 2.0 ** -150 * np.sqrt(f.size)
