@@ -202,6 +202,7 @@ bool launch_window_fixed(const Geom& g, const DevPtrs& p, int splits, cudaStream
 // 3D FP32 HOFKS at a shape the tile kernel is compiled for (dvm_kinetic_shapes.cu)
 bool tile3_shape(const Geom& g);
 bool fixed_shapes_on();  // (DVM_FIXED_SHAPES)
+bool window_eligible(const Geom& g);  // the per-thread windows can run g
 // the pass with CTA-shared source rows (dvm_kinetic_shared.cu)
 bool shared_eligible(const Geom& g);
 int shared_splits(const Geom& g, int sms);

@@ -266,6 +266,7 @@ __global__ void __launch_bounds__(256) k_window_fold_p(Geom g, DevPtrs p) {
   for (int q = 0; q < 3; ++q) wg[q * nc + c] = o[q];
 }
 
+}  // namespace
 
 bool window_eligible(const Geom& g) {
   if (g.d < 2 || g.precision == DVM_F64 || g.p != 1) return false;
@@ -276,6 +277,8 @@ bool window_eligible(const Geom& g) {
   const int Y = win_y(g.d);
   return g.nv[1] % Y == 0 && g.nv[0] % win_warps(g.d) == 0 && g.nx[1] >= Y && g.nc < (1LL << 31);
 }
+
+namespace {
 
 int sm_count() {
   static int n = 0;

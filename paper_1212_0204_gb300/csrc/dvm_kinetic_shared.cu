@@ -94,10 +94,10 @@ __global__ void __launch_bounds__(256) k_shared_fold(Geom g, DevPtrs p) {
   }
 }
 
-template <typename TS, int D, int FORM, bool P1, bool OUT>
+template <typename TS, int D, int FORM, bool P1, bool OUT, bool FLUSH = false>
 void launch_one(const Geom& g, const DevPtrs& p, int splits, cudaStream_t s, bool prepare) {
   constexpr int MINB = sizeof(TS) == 8 ? 2 : (FORM == kFormFks ? 4 : 3);
-  auto* k = k_kpass_shared<TS, D, FORM, P1, OUT, MINB>;
+  auto* k = k_kpass_shared<TS, D, FORM, P1, OUT, FLUSH, MINB>;
   const SharedLaunch sl = shape_of(g, splits);
   if (prepare) {
     // the most any configuration takes, so that handles do not lower it for
@@ -114,6 +114,11 @@ void launch_one(const Geom& g, const DevPtrs& p, int splits, cudaStream_t s, boo
 template <typename TS, int D, int FORM>
 void launch_form(const Geom& g, const DevPtrs& p, int splits, cudaStream_t s, bool prepare) {
   const bool out = any_outflow(g);
+  if constexpr (sizeof(TS) != 8)
+    if (window_eligible(g)) {
+      launch_one<TS, D, FORM, true, false, true>(g, p, splits, s, prepare);
+      return;
+    }
   if constexpr (FORM == kFormP) {
     launch_one<TS, D, FORM, true, false>(g, p, splits, s, prepare);  // periodic, p = 1
   } else {
