@@ -407,7 +407,8 @@ void launch_generic(const Geom& g, const DevPtrs& p, cudaStream_t s) {
 
 // Where both the per-thread windows and the shared rows can run (periodic, p = 1,
 // velocity counts a multiple of the windows'), per step in us, windows / shared.
-// 2D: FKS shared (256^2 x 32^2 173 / 158, 200^2 x 24^2 114 / 70); HOFKS windows, for
+// 2D: FKS shared (256^2 x 32^2 173 / 158, 200^2 x 24^2 114 / 70) unless few of the rows
+// are useful (2048 x 17 x 24^2 83 / 96); HOFKS windows, for
 // the shared rows' CTAs leave the Euler sub-steps beside them less room (256^2 x
 // 32^2 203 / 271, 512^2 x 32^2 873 / 991).
 // 3D: by the share of useful lanes, N_x of 32-wide rows against N_y of 16-row
@@ -421,7 +422,10 @@ void launch_generic(const Geom& g, const DevPtrs& p, cudaStream_t s) {
 // tile kernel's shapes stay with 1.
 static bool shared_faster(const Geom& g) {
   const bool fks = g.scheme == DVM_FKS, f32 = g.precision == DVM_F32;
-  if (g.d == 2) return fks;
+  if (g.d == 2) {
+    const long long bx = (g.nx[0] + 31LL) / 32 * 32, by = (g.nx[1] + 15LL) / 16 * 16, b4 = (g.nx[1] + 3LL) / 4 * 4;
+    return fks && 10 * bx * b4 >= 7 * g.nx[0] * by;
+  }
   if (!fks && (!f32 || tile3_shape(g))) return false;
   if (g.nc < (1 << 14)) return false;
   const long long bx = (g.nx[0] + 31LL) / 32 * 32, by = (g.nx[1] + 15LL) / 16 * 16;
@@ -429,17 +433,40 @@ static bool shared_faster(const Geom& g) {
   return g.nx[0] == bx && g.nx[1] == by && (g.nv[1] >= 16 || (fks && f32));
 }
 
+// Where the shared rows leave more threads without a cell than they save (small
+// planes: 32 columns of 16 rows a CTA), per step in us, per cell / shared:
+// 3D below 0.35 of the threads 8^3 x 16^3 FKS 120 / 185, outflow 101 / 198; 12^3 x 13^3
+// 71 / 83.  From 4096 cells up, or with more velocity pairs than twice the splits, so that a
+// CTA walks several in sequence: FP64 below a half (14^3 x 16^3 HOFKS 0.89 of the time of
+// the shared rows, 20^3 x 9^3 0.76), with outflow, whose rows beyond the domain cost the
+// shared rows more, below 0.56 (16^3 x 16^3 0.78, 20^3 0.75; 24^3, 0.5625 of the threads,
+// alike).  2D: first-order
+// outflow below 1000 cells (25^2 x 30^2 47 / 62, 16^2 x 21^2 37 / 44); HOFKS waits for the
+// Euler sub-steps there.
+static bool cell_faster(const Geom& g) {
+  bool out = false;
+  for (int i = 0; i < g.d; ++i) out |= g.bc[i] == DVM_BC_OUTFLOW;
+  const bool f64 = g.precision == DVM_F64;
+  if (g.d == 2) return out && !f64 && g.scheme == DVM_FKS && g.nc < 1000;
+  const long long columns = g.nx[0] * ((g.nx[1] + 15LL) / 16);
+  const long long cells = (long long)g.nx[0] * g.nx[1], threads = (columns + 31) / 32 * 32 * 16;
+  if (100 * cells < 35 * threads) return true;
+  if (g.nv[0] * g.nv[2] <= 100 && g.nc < 4096) return false;
+  return f64 ? 2 * cells < threads : out && 100 * cells < 56 * threads;
+}
+
 // Which kernel of the pass: 0 one thread per cell, 1 the per-thread windows
 // (and the kernels compiled for the configured shapes), 2 the CTA-shared rows.
 // The learned path keeps 1, which skips CTAs of flagged cells.  What 1 does not
-// take runs 2 where its columns are at least half filled; per cell against it:
+// take runs 2 where its columns are at least half filled and cell_faster does not
+// say otherwise; per cell against it:
 // 200^2 x 21^2 HOFKS 245 against 141 us, 60^3 x 13^3 5.2 against 1.82 ms, implosion
 // 300^2 x 36^2 (p = 2) 1.14 against 0.62 ms, FP64 256^2 x 32^2 5.06 against 3.85 ms.
 // 3D HOFKS without the learned path runs 1 only with the linear-term slice (its
 // single-quadratic form leaves these moments out): beyond the slice's launch
 // limits it is 2 or 0.
 static int kernel_of(const Geom& g) {
-  const bool sh = shared_eligible(g);
+  const bool sh = shared_eligible(g) && !cell_faster(g);
   const bool w = window_eligible(g) && (g.d == 2 || g.scheme == DVM_FKS || g.learn || linear_moments_fit(g));
   if (!w || !sh) return w ? 1 : (sh ? 2 : 0);
   return !g.learn && shared_faster(g) ? 2 : 1;
@@ -486,11 +513,15 @@ int kinetic_route(const Geom& g, int* rows) {
 bool kinetic_skips_deep(const Geom& g) { return kernel_of(g) == 1 && !getenv_generic(); }
 
 // 3D HOFKS: the single-quadratic form, whose linear-term moments need a
-// periodic box, integer shifts and a grid within the launch limits.
+// periodic box, integer shifts and a grid within the launch limits.  The shared rows
+// take it from 2^24 points up: below, the three passes of the linear term cost more
+// than the second quadratic (20^3 x 9^3 1.2, 16^3 x 13^3 1.17 times the step; 20^3 x 13^3, 18 M
+// points, 0.93).
 bool kinetic_linear_slice(const Geom& g) {
   if (g.d != 3 || g.scheme == DVM_FKS || g.p != 1 || !kinetic_is_windowed(g)) return false;
   for (int i = 0; i < 3; ++i)
     if (g.bc[i] != DVM_BC_PERIODIC) return false;
+  if (kernel_of(g) == 2 && g.nc * g.nvel < (1LL << 24)) return false;
   return linear_moments_fit(g);
 }
 
