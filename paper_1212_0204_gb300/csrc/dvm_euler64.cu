@@ -13,7 +13,7 @@
 // halved split fluxes g = (F +- alpha W) / 2 the limited slope of Eq. discmom
 // enters as a b / (a + b), saving the constants.  About 330 FP64 instructions
 // per cell and sub-step against 720 in the two-phase kernel.  A kinetic step's
-// sub-steps: 2D 256^2 1981 -> 901 us, 100^2 with 100 sub-steps 3184 -> 1317 us,
+// sub-steps: 2D 256^2 1981 -> 978 us, 100^2 with 100 sub-steps 3184 -> 1317 us,
 // 1D 200 cells (9 sub-steps) 195 -> 98 us.
 #include <math.h>
 

@@ -460,8 +460,8 @@ static bool cell_faster(const Geom& g) {
 // The learned path keeps 1, which skips CTAs of flagged cells.  What 1 does not
 // take runs 2 where its columns are at least half filled and cell_faster does not
 // say otherwise; per cell against it:
-// 200^2 x 21^2 HOFKS 245 against 141 us, 60^3 x 13^3 5.2 against 1.82 ms, implosion
-// 300^2 x 36^2 (p = 2) 1.14 against 0.62 ms, FP64 256^2 x 32^2 5.06 against 3.85 ms.
+// 200^2 x 21^2 HOFKS 217 against 146 us, 60^3 x 13^3 6.2 against 2.1 ms, implosion
+// 300^2 x 36^2 (p = 2) 1.7 against 0.54 ms, FP64 256^2 x 32^2 4.45 against 2.75 ms.
 // 3D HOFKS without the learned path runs 1 only with the linear-term slice (its
 // single-quadratic form leaves these moments out): beyond the slice's launch
 // limits it is 2 or 0.

@@ -170,9 +170,9 @@ bool shared_eligible(const Geom& g) {
 // waits for the 1/p as many Euler sub-steps beside it and the CTAs take their
 // SMs; 2D FP32 at least pairs / kShRun, for a split's sums are FP32 and the splits
 // are added in FP64.  Step of the implosion 200^2 x 30^2, c = 5, 8, 15, 30: 339, 287, 253, 260
-// us; FKS 200^2 x 20^2, c = 4, 7, 12: 65, 54, 63 us; FP64 HOFKS 100^2 x 40^2,
-// c = 10, 20, 40: 1471, 1163, 1124 us; HOFKS 64^2 x 25^2, c = 6, 12, 25: 126,
-// 135, 138 us.
+// us (with every value beyond the domain addressed by itself; 207 us at c = 10 since); FKS
+// 200^2 x 20^2, c = 4, 7, 12: 65, 54, 63 us; FP64 HOFKS 100^2 x 40^2, c = 10, 20, 40:
+// 1471, 1163, 1124 us; HOFKS 64^2 x 25^2, c = 6, 12, 25: 126, 135, 138 us.
 int shared_splits(const Geom& g, int sms) {
   const long long tiles = ((long long)g.nx[0] * ((g.nx[1] + kShTY - 1) / kShTY) + 31) / 32 * g.nx[2];
   const int pairs = g.nv[0] * g.nv[2];
